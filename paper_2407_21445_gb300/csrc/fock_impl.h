@@ -3,8 +3,10 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/fock.h"
@@ -157,6 +159,7 @@ struct Tier {
   int cb = 0, ck = 0;   // bra class, ket class
   bool reg = false;     // on the per-class register kernels (else the group kernels)
   bool r32 = false;     // group tier whose FP32 part runs on the FP32 register kernel
+  bool in_range = true;  // seeds within the FP32 exponent range, see seeds_in_range
   int tag = 0;          // class pair + 1 when class pairs are timed apart (tuning)
   int G = 1;            // lanes per quartet (group kernels)
   GroupConfig grp, g32;  // group kernels: FP64 and two-float lists; FP32 list (mixed)
@@ -172,6 +175,22 @@ struct Tier {
   int nunits;
   Unit *d_units;
 };
+
+// Whether the seeds pref (-2 alpha)^m F_m(T), pref = 1/sqrt(zeta + eta), m = 0..L,
+// of a class pair fit the FP32 exponent range for all exponents zeta in
+// [z0, z1], eta in [e0, e1] (sums of two primitive exponents), alpha = zeta eta /
+// (zeta + eta).  The powers pref (2 alpha)^m are formed before they meet F_m, and
+// the recursion makes nothing larger of them, so 2^120 leaves it room below
+// 2^128.  At the lower end F_m(0) = 1/(2m+1) counts, and the remainder of a value
+// (2^-48 of it) has to be a multiple of 2^-149: 2^-100.  With equal exponents
+// that admits f shells of 1.7e-3 .. 690, (fd|fd) of 5e-4 .. 3e3, (dd|dd) of 8e-5 ..
+// 3e4; outside a class pair runs in FP64 alone.
+inline bool seeds_in_range(int L, double z0, double z1, double e0, double e1) {
+  const double a0 = 2.0 * z0 / (z0 + e0) * e0, a1 = 2.0 * z1 / (z1 + e1) * e1;
+  const double hi = -0.5 * log2(z0 + e0) + L * std::max(0.0, log2(a1));
+  const double lo = -0.5 * log2(z1 + e1) + L * std::min(0.0, log2(a0)) - log2(2.0 * L + 1.0);
+  return hi < 120.0 && lo > -100.0;
+}
 
 // Threads that keep the chip busy: 152 SMs x 16 warps.
 constexpr long long kFillThreads = 152 * 16 * 32;
@@ -221,7 +240,7 @@ struct fock_shellpairs {
   int decay_nbins = 0;                // 0.5-bohr distance bins of the decay fit
   unsigned long long serial = 0;      // unique id (batch plan cache key)
   float gmax2 = 0.0f;                 // largest G_ab^2
-  bool ff_ok = false;                 // exponents and centres within the two-float range
+  bool ff_ok = false;                 // exponents, centres and integrals within the two-float range
   // device allocations
   void *d_block = nullptr;            // one allocation holding all pair arrays
   fk::DevPairs dev{};

@@ -555,7 +555,7 @@ cudaError_t launch_jk_tier(const Tier &t, const DevPairs &dp, const double *D, c
   a.fp32_cutoff = Df ? fp32_cutoff : 0.0;
   a.fp32_cutoff_f = (float)a.fp32_cutoff;
   a.Df = Df;
-  a.dmax = dp.E2 ? cp.dmax : nullptr;
+  a.dmax = dp.E2 && t.in_range ? cp.dmax : nullptr;
   a.gmax2 = cp.gmax2;
   set_screen_args(a, tau, Dshf, prim_eps, cp);
   return launch_tier(t, a, counters, st, par, index);
@@ -576,7 +576,7 @@ cudaError_t launch_jk_tier_batch(const Tier &t, const DevPairs &dp, const MolEnt
   a.mt = mt;
   a.fp32_cutoff = fp32_cutoff;
   a.fp32_cutoff_f = (float)a.fp32_cutoff;
-  a.dmax = dp.E2 ? dmax : nullptr;
+  a.dmax = dp.E2 && t.in_range ? dmax : nullptr;
   set_screen_args(a, tau, Dshf, prim_eps);
   return launch_tier(t, a, counters, st, par, index);
 }

@@ -1,0 +1,115 @@
+"""Edges of the two-float window of the J/K build: exponents on both sides of
+the limits that keep the seeds pref (-2 alpha)^m F_m of a class pair inside the
+FP32 exponent range, density elements far below the largest one, and handles
+in and out of the range in one batch.
+
+Tolerance of a default FP64 build: a primitive quartet in the window is below
+line = 2^-13 max(G_ab)^2 max|D| and held to 2^-40 of itself (2^-44 with four bits
+for the cancellation in the recursion), at most n^2 of them add up in an
+element; everything else is FP64 and held to 2^-44 of the largest element."""
+import numpy as np
+import pytest
+
+import molgen
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+TOL_MIXED = 1e-7
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA GPU required")
+    import paper_2407_21445_gb300 as fk
+    return torch, fk
+
+
+def _build(env, bas, D, tau, **kw):
+    torch, fk = env
+    b = fk.JKBuilder(bas, tau, fk.make_opts(**kw))
+    J, K = b.build(torch.tensor(D, device="cuda"))
+    torch.cuda.synchronize()
+    assert fk.fock_stream_status() == 0
+    b.close()
+    return J.cpu().numpy(), K.cpu().numpy()
+
+
+def _tolerance(bas, D, Jo, Ko):
+    gmax = float(np.max(oracle.schwarz(bas)[0]))
+    line = 2.0 ** -13 * gmax ** 2 * np.abs(D).max()
+    return len(D) ** 2 * line * 2.0 ** -40 + 2.0 ** -44 * max(np.abs(Jo).max(), np.abs(Ko).max())
+
+
+def _one_exponent(ls, a, small, spread=1.0):
+    """An s shell of exponent 1 with D = 1 and shells `ls` of exponent `a` within
+    `spread` of their radius with D = `small` times random numbers: their quartets
+    among themselves lie in the two-float window."""
+    rng = np.random.Generator(np.random.PCG64(720))
+    shells = [(0, np.zeros(3), [1.0], [1.0])]
+    shells += [(l, spread / np.sqrt(a) * rng.uniform(-1, 1, 3), [a], [1.0]) for l in ls]
+    bas = molgen.single_shell_basis(shells)
+    n = oracle.nbf(bas)
+    D = small * rng.uniform(-1, 1, (n, n))
+    D = 0.5 * (D + D.T)
+    D[0, 0] = 1.0
+    return bas, D
+
+
+# With one exponent a on every shell the limits 2^120 and 2^-100 of the seeds lie
+# at 690 and 1.7e-3 for (ff|ff), at 3200 and 5e-4 for (fd|fd); (dd|dd) ends at
+# 1e4 by the limit of the exponents themselves.
+RANGE = [([3, 3], a) for a in (2e-4, 1.5e-3, 3e-3, 600.0, 900.0, 2000.0, 5000.0)]
+RANGE += [([3, 2], a) for a in (4e-4, 1e-3, 1500.0, 2500.0, 9000.0)]
+RANGE += [([2, 2], a) for a in (2e-4, 9e3, 1.1e4)]
+
+
+@pytest.mark.parametrize("spread", [0.0, 1.0])
+@pytest.mark.parametrize("ls,a", RANGE)
+def test_exponents_at_the_edges(env, ls, a, spread):
+    bas, D = _one_exponent(ls, a, 1e-4, spread)
+    Jo, Ko = oracle.jk(bas, D, 1e-10)
+    J, K = _build(env, bas, D, 1e-10)
+    tol = _tolerance(bas, D, Jo, Ko)
+    assert np.abs(J - Jo).max() <= tol and np.abs(K - Ko).max() <= tol
+
+
+@pytest.mark.parametrize("group", [0, 8])
+@pytest.mark.parametrize("exps", [(1e-3, 1e3), (2e-3, 3.0), (1.0, 5e3)])
+def test_exponents_of_several_sizes(env, exps, group):
+    """Contracted f, d and p shells that hold tight and diffuse primitives."""
+    rng = np.random.Generator(np.random.PCG64(721))
+    shells = [(0, np.zeros(3), [1.0], [1.0])]
+    shells += [(l, 0.3 * rng.uniform(-1, 1, 3), list(exps), [0.6, 0.4]) for l in (3, 2, 1, 3)]
+    bas = molgen.single_shell_basis(shells)
+    n = oracle.nbf(bas)
+    D = 1e-4 * rng.uniform(-1, 1, (n, n))
+    D = 0.5 * (D + D.T)
+    D[0, 0] = 1.0
+    Jo, Ko = oracle.jk(bas, D, 1e-10)
+    J, K = _build(env, bas, D, 1e-10, group_override=group)
+    tol = _tolerance(bas, D, Jo, Ko)
+    assert np.abs(J - Jo).max() <= tol and np.abs(K - Ko).max() <= tol
+
+
+def test_batch_with_one_handle_out_of_range(env):
+    """A batch whose handles lie inside, partly outside (f pairs only) and wholly
+    outside the two-float range gives what each handle gives."""
+    torch, fk = env
+    mols = [_one_exponent([3, 2], 5.0, 1e-4), _one_exponent([3, 3], 5e3, 1e-4), _one_exponent([1, 2], 1e8, 1e-4)]
+    for pick in ([0, 1], [0, 1, 2]):
+        bs = [fk.JKBuilder(mols[i][0], 1e-10) for i in pick]
+        D = [torch.tensor(mols[i][1], device="cuda") for i in pick]
+        J, K = [torch.full_like(d, float("nan")) for d in D], [torch.full_like(d, float("nan")) for d in D]
+        fk.fock_build_jk_batched([b.handle for b in bs], D, 1e-10, J, K)
+        torch.cuda.synchronize()
+        assert fk.fock_stream_status() == 0
+        for i, j, k in zip(pick, J, K):
+            bas, Dn = mols[i]
+            Jo, Ko = oracle.jk(bas, Dn, 1e-10)
+            tol = _tolerance(bas, Dn, Jo, Ko)
+            assert np.abs(j.cpu().numpy() - Jo).max() <= tol and np.abs(k.cpu().numpy() - Ko).max() <= tol
+        for b in bs:
+            b.close()
