@@ -113,3 +113,18 @@ def test_batch_with_one_handle_out_of_range(env):
             assert np.abs(j.cpu().numpy() - Jo).max() <= tol and np.abs(k.cpu().numpy() - Ko).max() <= tol
         for b in bs:
             b.close()
+
+
+def test_fp32_overflow_shows(env):
+    """FP32 quartets whose digested value passes the largest FP32 number: the
+    element is infinite or NaN, never a finite wrong number."""
+    torch, fk = env
+    rng = np.random.Generator(np.random.PCG64(723))
+    bas = molgen.random_shells(rng, [0, 1, 2, 3], spread=0.5, kmax=2)
+    D = np.full((oracle.nbf(bas),) * 2, 3e38)
+    Jo, Ko = oracle.jk(bas, D, 1e-10)
+    J, K = _build(env, bas, D, 1e-10, precision=fk.FOCK_MIXED, fp32_cutoff=1e300)
+    assert not (np.isfinite(J).all() and np.isfinite(K).all())
+    for x, xo in ((J, Jo), (K, Ko)):
+        ok = np.isfinite(x)
+        assert np.abs(x - xo)[ok].max(initial=0.0) <= 1e-4 * np.abs(xo).max()
