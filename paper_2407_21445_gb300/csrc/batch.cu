@@ -201,7 +201,7 @@ fock_status build_plan(const fock_shellpairs *const *bases, int nmol, BatchPlan 
   bp->dev.nbf = 0;  // per molecule, from the table
   for (size_t t = 0; t < bp->tiers.size(); ++t) {
     bp->tiers[t].d_units = d_units + first[t];
-    ce = configure_tier(bp->tiers[t], bp->ff_ok && bp->tiers[t].in_range, bp->mixed);
+    ce = configure_tier(bp->tiers[t], bp->ff_ok, bp->mixed);
     if (ce != cudaSuccess) {
       delete bp;
       return batch_status(ce);

@@ -334,7 +334,8 @@ cudaError_t launch_symmetrize_batch(const MolEntry *mt, const long long *n2_pref
 cudaError_t launch_jk_tier_batch(const Tier &t, const DevPairs &dp, const MolEntry *mt, const double *Dsh,
                                  const float *Dshf, const unsigned *dmax, double tau, double prim_eps,
                                  int *counters, cudaStream_t st, StreamSet *par, int index, double fp32_cutoff);
-// Launch shapes of a tier's kernels; ff: the two-float path is on.
+// Launch shapes of a tier's kernels; ff: the two-float path is on, mixed: the FP32
+// path (both only for a tier in range).
 cudaError_t configure_tier(Tier &t, bool ff, bool mixed);
 int read_and_clear_status(cudaStream_t st, int *status);
 int read_bounds(long long out[2]);

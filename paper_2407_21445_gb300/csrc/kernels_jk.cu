@@ -452,6 +452,8 @@ cudaError_t launch_symmetrize(double *J, double *K, int n, cudaStream_t st) {
 
 cudaError_t configure_tier(Tier &t, bool ff, bool mixed) {
   cudaError_t e = cudaSuccess;
+  ff = ff && t.in_range;
+  mixed = mixed && t.in_range;
   int dev = 0, nsm = 0, per_sm = 0, warps = 4;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -552,7 +554,7 @@ cudaError_t launch_jk_tier(const Tier &t, const DevPairs &dp, const double *D, c
   a.tau = tau;
   a.J = J;
   a.K = K;
-  a.fp32_cutoff = Df ? fp32_cutoff : 0.0;
+  a.fp32_cutoff = Df && t.in_range ? fp32_cutoff : 0.0;
   a.fp32_cutoff_f = (float)a.fp32_cutoff;
   a.Df = Df;
   a.dmax = dp.E2 && t.in_range ? cp.dmax : nullptr;
@@ -574,7 +576,7 @@ cudaError_t launch_jk_tier_batch(const Tier &t, const DevPairs &dp, const MolEnt
   a.Dsh = Dsh;
   a.tau = tau;
   a.mt = mt;
-  a.fp32_cutoff = fp32_cutoff;
+  a.fp32_cutoff = t.in_range ? fp32_cutoff : 0.0;
   a.fp32_cutoff_f = (float)a.fp32_cutoff;
   a.dmax = dp.E2 && t.in_range ? dmax : nullptr;
   set_screen_args(a, tau, Dshf, prim_eps);

@@ -115,6 +115,41 @@ def test_batch_with_one_handle_out_of_range(env):
             b.close()
 
 
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("group", [0, 4])
+@pytest.mark.parametrize("ls,a", [([3, 3], 2e-4), ([3, 3], 600.0), ([3, 2], 2000.0), ([3, 3], 5000.0), ([2, 2], 5e4)])
+def test_mixed_exponents_at_the_edges(env, ls, a, group, batched):
+    """Mixed builds whose f and d quartets lie below the FP32 cutoff: where the
+    seeds would leave the FP32 exponent range the class pair runs in FP64."""
+    torch, fk = env
+    bas, D = _one_exponent(ls, a, 1e-8)
+    Jo, Ko = oracle.jk(bas, D, 1e-13)
+    opts = dict(precision=fk.FOCK_MIXED, group_override=group)
+    if batched:
+        b = fk.JKBuilder(bas, 1e-13, fk.make_opts(**opts))
+        Dt = torch.tensor(D, device="cuda")
+        J, K = torch.empty_like(Dt), torch.empty_like(Dt)
+        fk.fock_build_jk_batched([b.handle], [Dt], 1e-13, [J], [K])
+        torch.cuda.synchronize()
+        J, K = J.cpu().numpy(), K.cpu().numpy()
+        b.close()
+    else:
+        J, K = _build(env, bas, D, 1e-13, **opts)
+    assert np.abs(J - Jo).max() <= TOL_MIXED and np.abs(K - Ko).max() <= TOL_MIXED
+
+
+def test_mixed_stats_out_of_range(env):
+    """No FP32 quartet is counted for a class pair that runs in FP64."""
+    torch, fk = env
+    bas, D = _one_exponent([3], 5000.0, 1e-8)
+    b = fk.JKBuilder(bas, 1e-13, fk.make_opts(precision=fk.FOCK_MIXED))
+    st = b.stats(D)
+    c = fk.JKBuilder(_one_exponent([3], 500.0, 1e-8)[0], 1e-13, fk.make_opts(precision=fk.FOCK_MIXED)).stats(D)
+    b.close()
+    assert st["quartets_evaluated"] == c["quartets_evaluated"]
+    assert st["quartets_fp32"] < c["quartets_fp32"]
+
+
 def test_fp32_overflow_shows(env):
     """FP32 quartets whose digested value passes the largest FP32 number: the
     element is infinite or NaN, never a finite wrong number."""
