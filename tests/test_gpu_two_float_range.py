@@ -115,6 +115,26 @@ def test_batch_with_one_handle_out_of_range(env):
             b.close()
 
 
+@pytest.mark.parametrize("log2_scale", [-24, -39, -41, -59])
+def test_small_elements_of_a_small_density(env, log2_scale):
+    """Densities whose elements spread over 2^-36 of the largest, on both sides of
+    the smallest max|D| that the window takes (2^-40): every element counts."""
+    rng = np.random.Generator(np.random.PCG64(722))
+    bas = molgen.random_shells(rng, [0, 1, 2, 0, 1, 3], spread=4.0, kmax=4)
+    n = oracle.nbf(bas)
+    sizes = [oracle.ncart(int(l)) for l in bas["l"]]
+    w = np.repeat(2.0 ** -np.array([0.0, 4.0, 8.0, 12.0, 16.0, 18.0]), sizes)
+    D = rng.uniform(-1, 1, (n, n)) * w[:, None] * w[None]
+    D = 0.5 * (D + D.T)
+    D[0, 0] = 1.0
+    D *= 2.0 ** log2_scale
+    tau = 1e-22 * 2.0 ** log2_scale
+    Jo, Ko = oracle.jk(bas, D, tau)
+    J, K = _build(env, bas, D, tau)
+    tol = 1e-10 * 2.0 ** log2_scale
+    assert np.abs(J - Jo).max() <= tol and np.abs(K - Ko).max() <= tol
+
+
 @pytest.mark.parametrize("batched", [False, True])
 @pytest.mark.parametrize("group", [0, 4])
 @pytest.mark.parametrize("ls,a", [([3, 3], 2e-4), ([3, 3], 600.0), ([3, 2], 2000.0), ([3, 3], 5000.0), ([2, 2], 5e4)])
