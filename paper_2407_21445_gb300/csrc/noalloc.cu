@@ -44,6 +44,7 @@ extern "C" fock_status fock_build_jk_noalloc(const fock_shellpairs *sp, const do
   const int ns = sp->nshell, n = sp->nbf;
   const size_t nt = sp->tiers.size();
   const bool mixed = sp->opts.precision == FOCK_MIXED && sp->opts.fp32_cutoff > 0.0;
+  RelaxedCaptureMode relaxed;
   const ScratchLayout L = scratch_layout(sp);  // the layout fock_build_jk uses
   const size_t cnt = L.df_off - L.cnt_off;     // counters, a multiple of 256
   if (L.total > kNoallocBytes + (cnt - 256) || L.total > kNoallocBytes + kNoallocTail)

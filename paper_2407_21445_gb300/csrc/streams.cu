@@ -71,9 +71,9 @@ StreamSet *lease_streams(cudaStream_t user) {
   for (int k = 0; k < kSets - 1; ++k) {
     StreamSet &s = sets[k];
     if (s.leased) continue;
-    bool idle = true;
-    for (int i = 0; i < kParStreams && idle && s.used; ++i) idle = cudaEventQuery(s.join[i]) == cudaSuccess;
-    if (!idle) {
+    cudaError_t q = cudaSuccess;
+    for (int i = 0; i < kParStreams && q == cudaSuccess && s.used; ++i) q = cudaEventQuery(s.join[i]);
+    if (q != cudaSuccess) {
       cudaGetLastError();  // cudaErrorNotReady
       continue;
     }

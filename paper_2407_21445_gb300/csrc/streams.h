@@ -23,10 +23,23 @@ struct StreamSet {
 // handle is built, so that a build itself creates nothing).
 cudaError_t init_streams();
 
+// Event queries and stream-ordered allocations on any stream are among the calls
+// that a global-mode capture (torch's default) forbids to every thread, and one
+// such call breaks the capture.  A build makes them on streams that no capture
+// sees; its thread is in relaxed mode meanwhile.
+struct RelaxedCaptureMode {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCaptureMode() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCaptureMode() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  RelaxedCaptureMode(const RelaxedCaptureMode &) = delete;
+  RelaxedCaptureMode &operator=(const RelaxedCaptureMode &) = delete;
+};
+
 // A set for one build on `user`, or null when the build has to stay on that one
 // stream: it is being captured, or every set is still busy with builds of other
 // streams (sharing a set with another stream's unfinished build would order
-// two streams that the caller keeps independent).
+// two streams that the caller keeps independent).  Called under a
+// RelaxedCaptureMode.
 StreamSet *lease_streams(cudaStream_t user);
 void return_streams(StreamSet *set);
 
