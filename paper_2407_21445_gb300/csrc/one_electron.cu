@@ -182,13 +182,15 @@ __global__ void __launch_bounds__(128) k_one_prims(OneArgs a) {
     const double X = Px - a.axyz[3 * c], Y = Py - a.axyz[3 * c + 1], Z = Pz - a.axyz[3 * c + 2];
     const double T = p * fma(X, X, fma(Y, Y, Z * Z));
     double F[L + 1];
-    const float Tf = d2f_small(T);  // grid decision on the FP32 units
-    if (Tf < (float)BOYS_TMAX) {
-      const int gi = __float2int_rn(Tf * (float)BOYS_INVH);
+    // decisions on the integer units, by the high word of T: T < 64 reads the
+    // table, T < 2^127 has an FP32 seed for the square root
+    const unsigned th = (unsigned)__double2hiint(T) & 0x7fffffffu;
+    if (th < 0x40500000u) {
+      const int gi = __float2int_rn(d2f_small(T) * (float)BOYS_INVH);
       const double x = (gi == 0 ? 0.0 : f2d_pos((float)gi * (float)BOYS_H)) - T;
       sfor<L + 1>([&](auto m) { F[FK_CI(m)] = boys_taylor(a.boys, gi, FK_CI(m), x); });
     } else {
-      const double rt = rsqrt_nh(T, Tf), it = rt * rt;
+      const double rt = th < 0x47e00000u ? rsqrt_nh(T, d2f_small(T)) : rsqrt(T), it = rt * rt;
       F[0] = 0.88622692545275801365 * rt;
       sfor<L>([&](auto m) { F[FK_CI(m) + 1] = F[FK_CI(m)] * ((FK_CI(m) + 0.5) * it); });
     }
