@@ -331,10 +331,24 @@ int blocks_for(long long n) {
   return (int)(b > 4096 ? 4096 : (b < 1 ? 1 : b));
 }
 
+// A grid has at most 65535 blocks of columns: wider layers take several launches.
+constexpr int kMaxCols = 65535 * BN;
 template <bool TB, int EPI>
-cudaError_t gemm(const GemmArgs &g, cudaStream_t st) {
-  k_gemm<TB, EPI><<<dim3((g.M + BM - 1) / BM, (g.N + BN - 1) / BN), GTHREADS, 0, st>>>(g);
-  return cudaGetLastError();
+cudaError_t gemm(GemmArgs g, cudaStream_t st) {
+  for (int left = g.N;; left -= kMaxCols) {
+    g.N = left < kMaxCols ? left : kMaxCols;
+    k_gemm<TB, EPI><<<dim3((g.M + BM - 1) / BM, (g.N + BN - 1) / BN), GTHREADS, 0, st>>>(g);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || left <= kMaxCols) return e;
+    // the next columns; rows keep their stride
+    g.B += TB ? (size_t)kMaxCols * g.ldb : (size_t)kMaxCols;
+    g.C += kMaxCols;
+    if (g.act) g.act += kMaxCols;
+    if (g.bias) g.bias += kMaxCols;
+    if (g.aux) g.aux += kMaxCols;
+    if (g.target) g.target += kMaxCols;
+    if (g.mask) g.mask += kMaxCols;
+  }
 }
 
 Bf16Map bf16_map(const fock_mlp *n) {
