@@ -79,6 +79,7 @@ bool same_opts(const fock_shellpairs *a, const fock_shellpairs *b) {
          a->opts.fp32_cutoff == b->opts.fp32_cutoff && a->opts.prune_eps == b->opts.prune_eps &&
          a->opts.group_override == b->opts.group_override && a->opts.warp_scratch == b->opts.warp_scratch &&
          a->opts.reg_max_L == b->opts.reg_max_L && a->opts.tune_isolate == b->opts.tune_isolate &&
+         a->opts.two_float == b->opts.two_float &&
          memcmp(a->opts.schedule, b->opts.schedule, sizeof(a->opts.schedule)) == 0 && a->device == b->device;
 }
 

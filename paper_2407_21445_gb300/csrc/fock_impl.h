@@ -240,7 +240,7 @@ struct fock_shellpairs {
   int decay_nbins = 0;                // 0.5-bohr distance bins of the decay fit
   unsigned long long serial = 0;      // unique id (batch plan cache key)
   float gmax2 = 0.0f;                 // largest G_ab^2
-  bool ff_ok = false;                 // exponents, centres and integrals within the two-float range
+  bool ff_ok = false;                 // two floats wanted; exponents, centres and integrals within their range
   // device allocations
   void *d_block = nullptr;            // one allocation holding all pair arrays
   fk::DevPairs dev{};

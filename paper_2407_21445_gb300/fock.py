@@ -41,7 +41,7 @@ class fock_opts(ctypes.Structure):
     _fields_ = [("precision", ctypes.c_int32), ("fp32_cutoff", ctypes.c_double), ("prune_eps", ctypes.c_double),
                 ("group_override", ctypes.c_int32), ("warp_scratch", ctypes.c_int32), ("reg_max_L", ctypes.c_int32),
                 ("tune_isolate", ctypes.c_int32), ("schedule", ctypes.c_int8 * (NCLASS * NCLASS)),
-                ("k_mode", ctypes.c_int32), ("k_thresh", ctypes.c_double)]
+                ("k_mode", ctypes.c_int32), ("k_thresh", ctypes.c_double), ("two_float", ctypes.c_int32)]
 
 
 _lock = threading.Lock()
@@ -179,8 +179,9 @@ class _BasisArrays:
 
 
 def make_opts(precision=FOCK_FP64, fp32_cutoff=1e-5, prune_eps=1e-3, group_override=0, warp_scratch=0,
-              reg_max_L=0, schedule=None, k_mode=0, k_thresh=5e-6) -> fock_opts:
+              reg_max_L=0, schedule=None, k_mode=0, k_thresh=5e-6, two_float=True) -> fock_opts:
     o = fock_opts()
+    o.two_float = 0 if two_float else -1
     o.k_mode = k_mode
     o.k_thresh = k_thresh
     o.reg_max_L = reg_max_L

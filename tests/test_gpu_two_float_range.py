@@ -135,6 +135,47 @@ def test_small_elements_of_a_small_density(env, log2_scale):
     assert np.abs(J - Jo).max() <= tol and np.abs(K - Ko).max() <= tol
 
 
+def test_large_density_element_far_away(env):
+    """One element of D is 2^30 times the others, on a shell too far away to
+    exchange with them: every contribution to the near shells' K lies in the
+    window (2^-40 of itself), or, with the window turned off, is FP64."""
+    torch, fk = env
+    rng = np.random.Generator(np.random.PCG64(724))
+    bas = molgen.random_shells(rng, [0, 0, 1, 2, 3, 1], spread=2.0, kmax=4)
+    bas["center"][0] = [0.0, 0.0, 90.0]
+    n = oracle.nbf(bas)
+    D = rng.uniform(-1, 1, (n, n))
+    D = 0.5 * (D + D.T)
+    D[0, :] = D[:, 0] = 0.0
+    D[0, 0] = 2.0 ** 30
+    Jo, Ko = oracle.jk(bas, D, 1e-12)
+    g2 = float(np.max(oracle.schwarz(bas)[0][1:, 1:])) ** 2
+    for two_float, rel in ((True, 2.0 ** -40), (False, 2.0 ** -46)):
+        J, K = _build(env, bas, D, 1e-12, two_float=two_float)
+        assert np.abs(J - Jo).max() <= 2.0 ** -44 * np.abs(Jo).max()
+        assert np.abs(K - Ko)[1:, 1:].max() <= n * n * g2 * rel
+
+
+def test_window_turned_off(env):
+    """two_float = -1: no launch of its own for two floats, and the same J and K."""
+    torch, fk = env
+    p = molgen.problem(0)
+    b = [fk.JKBuilder(p.basis, p.tau, fk.make_opts(two_float=t)) for t in (True, False)]
+    assert fk.fock_kernels_per_build(b[1].handle) < fk.fock_kernels_per_build(b[0].handle)
+    D = torch.tensor(p.D, device="cuda")
+    (J0, K0), (J1, K1) = (x.build(D) for x in b)
+    assert float((J0 - J1).abs().max()) <= 1e-10 and float((K0 - K1).abs().max()) <= 1e-10
+    with pytest.raises(fk.FockError):  # one choice per batch
+        fk.fock_build_jk_batched([x.handle for x in b], [D, D], p.tau, [J0, J1], [K0, K1])
+    for v in (1, -2):
+        o = fk.make_opts()
+        o.two_float = v
+        with pytest.raises(fk.FockError):
+            fk.JKBuilder(p.basis, p.tau, o)
+    for x in b:
+        x.close()
+
+
 @pytest.mark.parametrize("batched", [False, True])
 @pytest.mark.parametrize("group", [0, 4])
 @pytest.mark.parametrize("ls,a", [([3, 3], 2e-4), ([3, 3], 600.0), ([3, 2], 2000.0), ([3, 3], 5000.0), ([2, 2], 5e4)])
