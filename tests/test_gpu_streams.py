@@ -58,3 +58,48 @@ def test_build_beside_a_global_capture(env, entry):
     torch.cuda.synchronize()
     assert _diff(out[0], ref) <= TOL
     b.close()
+
+
+def test_more_streams_than_sets(env):
+    """Builds of four streams in flight together, more than the pool has sets: the
+    others run on the caller's stream alone and give the same."""
+    torch, fk = env
+    p = molgen.problem(1, carbons=10)
+    b = fk.JKBuilder(p.basis, p.tau)
+    scale = (1.0, 0.5, -2.0, 3.0)
+    D = [torch.tensor(s * p.D, device="cuda") for s in scale]
+    ref = [b.build(d) for d in D]  # each its own: the screening weighs the density
+    out = [tuple(torch.full_like(D[0], float("nan")) for _ in range(2)) for _ in D]
+    streams = [torch.cuda.Stream() for _ in D]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for d, o, s in zip(D, out, streams):
+            b.build(d, *o, stream=s)
+    torch.cuda.synchronize()
+    for o, r in zip(out, ref):
+        assert _diff(o, r) <= TOL
+    b.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_captured_build_writes_both_matrices(env, precision):
+    """J and K are both rewritten by every replay, from the density it finds."""
+    torch, fk = env
+    p = molgen.problem(1, carbons=4)
+    b = fk.JKBuilder(p.basis, p.tau, fk.make_opts(precision=precision))
+    D = torch.tensor(p.D, device="cuda")
+    J, K = torch.empty_like(D), torch.empty_like(D)
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        b.build(D, J, K, stream=s)
+    for scale in (1.0, 0.25):
+        D.copy_(torch.tensor(scale * p.D))
+        ref = b.build(D)
+        J.fill_(float("nan"))
+        K.fill_(float("nan"))
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert _diff((J, K), ref) <= (TOL if precision == 0 else 1e-7)
+    b.close()
