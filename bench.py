@@ -39,6 +39,8 @@ UNIT = "ERI/s"
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # FP32 (FFMA) peak: 152 SMs x 128 lanes x 2 flop x 2.07 GHz.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
+# the same units at ten instructions per multiply-add of two floats
+TWO_FLOAT_PEAK_TFLOPS = FP32_PEAK_TFLOPS / 10
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -311,17 +313,34 @@ def max_over_ranks(ms: float, dist, dev) -> float:
     return float(t.item())
 
 
+def pipe_work(windows):
+    """Modelled operations of a build (JKBuilder.window_stats of one or of
+    several molecules) as mixed_peak_frac takes them."""
+    f64, ff, f32 = (sum(w[k] for w in windows) for k in ("flops_fp64", "flops_two_float", "flops_fp32"))
+    return {"flops_model": f64 + ff + f32, "flops_model_fp32": f32, "flops_two_float": ff}
+
+
+def work_shares(st):
+    n = max(1.0, st["flops_model"])
+    return {"fp32_flop_share": st["flops_model_fp32"] / n, "two_float_flop_share": st["flops_two_float"] / n}
+
+
 def mixed_peak_frac(st, ms):
-    """Roofline of the mixed path: the modelled FP64 and FP32 operations each
-    over their own pipe's peak; `combined` = the fraction of the build time
-    the two pipes would need at peak."""
+    """Roofline of a build by arithmetic: the modelled operations in FP64, in
+    two floats and in FP32, each over the peak of the units that run them
+    (two floats: ten FP32 instructions per multiply-add); `combined` = the
+    fraction of the build time that they would need at peak one after the other
+    (FP64 and FP32 units work side by side, so that it can pass 1)."""
     t = ms * 1e-3
-    f32 = st["flops_model_fp32"]
-    f64 = st["flops_model"] - f32
-    a64, a32 = f64 / t / 1e12, f32 / t / 1e12
-    return {"fp64_achieved_tflops": a64, "fp64_frac": a64 / FP64_PEAK_TFLOPS, "fp32_achieved_tflops": a32,
-            "fp32_frac": a32 / FP32_PEAK_TFLOPS, "combined": a64 / FP64_PEAK_TFLOPS + a32 / FP32_PEAK_TFLOPS,
-            "peaks_tflops": {"fp64": FP64_PEAK_TFLOPS, "fp32": FP32_PEAK_TFLOPS}}
+    f32, ff = st["flops_model_fp32"], st.get("flops_two_float", 0.0)
+    f64 = st["flops_model"] - f32 - ff
+    a64, aff, a32 = f64 / t / 1e12, ff / t / 1e12, f32 / t / 1e12
+    return {"fp64_achieved_tflops": a64, "fp64_frac": a64 / FP64_PEAK_TFLOPS,
+            "two_float_achieved_tflops": aff, "two_float_frac": aff / TWO_FLOAT_PEAK_TFLOPS,
+            "fp32_achieved_tflops": a32, "fp32_frac": a32 / FP32_PEAK_TFLOPS,
+            "combined": a64 / FP64_PEAK_TFLOPS + aff / TWO_FLOAT_PEAK_TFLOPS + a32 / FP32_PEAK_TFLOPS,
+            "peaks_tflops": {"fp64": FP64_PEAK_TFLOPS, "two_float": TWO_FLOAT_PEAK_TFLOPS,
+                             "fp32": FP32_PEAK_TFLOPS}}
 
 
 def tuned(args, fk, bases, Ds, tau, prec):
@@ -379,6 +398,7 @@ def batched_leg(args, fk, torch, dev, stream, flush, nmol, steps, warmup, e2e_st
 
     bs = setup(fk.FOCK_FP64)
     stats = [b.stats(p.D) for b, p in zip(bs, probs)]
+    work = pipe_work([b.window_stats(p.D) for b, p in zip(bs, probs)])
     eris = sum(s["eris_schwarz"] for s in stats)
     flops = sum(s["flops_model"] for s in stats)
     ms = float(np.mean(run(bs)))
@@ -412,6 +432,7 @@ def batched_leg(args, fk, torch, dev, stream, flush, nmol, steps, warmup, e2e_st
         b.close()
     mbs = setup(fk.FOCK_MIXED)
     mst = [b.stats(p.D) for b, p in zip(mbs, probs)]
+    mwork = pipe_work([b.window_stats(p.D) for b, p in zip(mbs, probs)])
     mms = float(np.mean(run(mbs)))
     err = max(max(float((j - jr).abs().max()), float((k - kr).abs().max()))
               for j, k, jr, kr in zip(Js, Ks, Jref, Kref))
@@ -419,8 +440,6 @@ def batched_leg(args, fk, torch, dev, stream, flush, nmol, steps, warmup, e2e_st
         b.close()
     q32 = sum(s["quartets_fp32"] for s in mst)
     q = sum(s["quartets_evaluated"] for s in mst)
-    f32 = sum(s["flops_model_fp32"] for s in mst)
-    mflops = sum(s["flops_model"] for s in mst)
     nbf = [p.nbf for p in probs]
     achieved = flops / (ms * 1e-3) / 1e12
     return {
@@ -429,12 +448,12 @@ def batched_leg(args, fk, torch, dev, stream, flush, nmol, steps, warmup, e2e_st
         "molecules": len(probs), "nbf_total": int(sum(nbf)), "nbf_min": int(min(nbf)), "nbf_max": int(max(nbf)),
         "schwarz_thresh": tau, "eris_per_step": int(eris), "steps": steps, "warmup": warmup,
         "fp64": {"ms_per_step": ms, "value": eris / (ms * 1e-3), "unit": UNIT, "achieved_tflops": achieved,
-                 "frac_of_fp64_peak": achieved / FP64_PEAK_TFLOPS, "schedule": tunes.get(fk.FOCK_FP64)},
+                 "frac_of_fp64_peak": achieved / FP64_PEAK_TFLOPS, "peak_frac": mixed_peak_frac(work, ms),
+                 "schedule": tunes.get(fk.FOCK_FP64)},
         "mixed": {"ms_per_step": mms, "value": eris / (mms * 1e-3), "unit": UNIT, "speedup_vs_fp64": ms / mms,
                   "fp32_cutoff": args.fp32_cutoff, "max_abs_diff_vs_fp64": err,
-                  "fp32_quartet_share": q32 / max(q, 1.0), "fp32_flop_share": f32 / max(mflops, 1.0),
-                  "schedule": tunes.get(fk.FOCK_MIXED),
-                  "peak_frac": mixed_peak_frac({"flops_model": mflops, "flops_model_fp32": f32}, mms)},
+                  "fp32_quartet_share": q32 / max(q, 1.0), **work_shares(mwork),
+                  "schedule": tunes.get(fk.FOCK_MIXED), "peak_frac": mixed_peak_frac(mwork, mms)},
         "_e2e_ms": e2e_ms, "_nbytes": nbytes, "_eris": eris, "_flops": flops,
     }
 
@@ -483,19 +502,19 @@ def alkane_leg(args, fk, torch, dev, stream, flush):
     ref = None
     for name, prec in (("fp64", fk.FOCK_FP64), ("mixed", fk.FOCK_MIXED)):
         b = fk.JKBuilder(p.basis, p.tau, fk.make_opts(precision=prec, fp32_cutoff=args.fp32_cutoff))
-        st = b.stats(p.D)
+        st, work = b.stats(p.D), pipe_work([b.window_stats(p.D)])
         ms = float(np.mean(time_steps(torch, dev, stream, flush, lambda: b.build(D, J, K), args.steps,
                                       max(3, args.warmup))))
         leg = {"ms_per_step": ms, "value": st["eris_schwarz"] / (ms * 1e-3), "unit": UNIT}
         if prec == fk.FOCK_FP64:
             ach = st["flops_model"] / (ms * 1e-3) / 1e12
-            leg.update(achieved_tflops=ach, frac_of_fp64_peak=ach / FP64_PEAK_TFLOPS)
+            leg.update(achieved_tflops=ach, frac_of_fp64_peak=ach / FP64_PEAK_TFLOPS,
+                       peak_frac=mixed_peak_frac(work, ms))
             ref = (ms, J.clone(), K.clone())
         else:
             leg.update(speedup_vs_fp64=ref[0] / ms,
                        max_abs_diff_vs_fp64=max(float((J - ref[1]).abs().max()), float((K - ref[2]).abs().max())),
-                       fp32_flop_share=st["flops_model_fp32"] / max(1.0, st["flops_model"]),
-                       peak_frac=mixed_peak_frac(st, ms))
+                       peak_frac=mixed_peak_frac(work, ms), **work_shares(work))
         out[name] = leg
         b.close()
     return out
@@ -746,7 +765,7 @@ def main():
     D = torch.tensor(p.D, device=dev, dtype=torch.float64)
     opts, tune = tuned(args, fk, [p.basis], [D], p.tau, prec)
     builder = fk.JKBuilder(p.basis, p.tau, opts)
-    st = builder.stats(p.D)
+    st, work = builder.stats(p.D), pipe_work([builder.window_stats(p.D)])
     nk = fk.fock_kernels_per_build(builder.handle)
     J = torch.empty_like(D)
     K = torch.empty_like(D)
@@ -806,7 +825,7 @@ def main():
     if not args.no_mixed_leg and args.precision == "fp64":
         mopts, mtune = tuned(args, fk, [p.basis], [D], p.tau, fk.FOCK_MIXED)
         mb = fk.JKBuilder(p.basis, p.tau, mopts)
-        mst = mb.stats(p.D)
+        mst, mwork = mb.stats(p.D), pipe_work([mb.window_stats(p.D)])
         builder.build(D, J, K)
         Jm = torch.empty_like(D)
         Km = torch.empty_like(D)
@@ -818,8 +837,8 @@ def main():
                  "speedup_vs_fp64": ms / mms, "fp32_cutoff": args.fp32_cutoff,
                  "max_abs_diff_vs_fp64": err, "trace_diff_vs_fp64": trd,
                  "fp32_quartet_share": mst["quartets_fp32"] / max(1.0, mst["quartets_evaluated"]),
-                 "fp32_flop_share": mst["flops_model_fp32"] / max(1.0, mst["flops_model"]), "schedule": mtune,
-                 "peak_frac": mixed_peak_frac(mst, mms), "steps": msteps, "warmup": 3}
+                 **work_shares(mwork), "schedule": mtune,
+                 "peak_frac": mixed_peak_frac(mwork, mms), "steps": msteps, "warmup": 3}
         mb.close()
 
     # ---- extra keys: C20H42 (FP64 and mixed) and a TZ batch up to f ---------
@@ -839,12 +858,13 @@ def main():
             "data": "synthetic", "config": dict(workload_config(p, st, args.precision), schedule=tune),
             "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": achieved / FP64_PEAK_TFLOPS,
+                         "by_arithmetic": mixed_peak_frac(work, ms),
                          "traffic": profile_traffic(kernel_hash()) if args.config == 2 else None,
                          "peak_note": "FP64 pipe, 152 SMs x 2 FMA/clk x 2.07 GHz = 1.2586 TFLOP/s (DFMA probe "
-                                      "1.256, profiles/fp64_fp32_peak.md); achieved = modelled FP64 flops of the "
-                                      "evaluated quartets / device time of the whole build (ERI kernels > 99.9 %); "
-                                      "most of these operations run as pairs of FP32 numbers on the FP32 units, so "
-                                      "that the fraction is a rate and can pass 1",
+                                      "1.256); achieved = modelled FP64 flops of the evaluated quartets / device "
+                                      "time of the whole build (ERI kernels > 99.9 %); most of these operations run "
+                                      "as pairs of FP32 numbers on the FP32 units, so that frac is a rate and can "
+                                      "pass 1: by_arithmetic divides them over the units that run them",
                          "traffic_note": "DRAM bytes of one FP64 build's launches (ncu, 1 pass, caches emptied "
                                          "before each launch: the pair data and tables are re-read per launch); "
                                          "algorithmic bytes D + J + K = 3 N^2 x 8 B"},

@@ -78,6 +78,8 @@ def lib() -> ctypes.CDLL:
             L.fock_build_jk_batched.restype = i
             L.fock_work_stats.argtypes = [p, p, d, p]
             L.fock_work_stats.restype = i
+            L.fock_window_stats.argtypes = [p, p, d, p]
+            L.fock_window_stats.restype = i
             L.fock_stream_status.argtypes = [p]
             L.fock_stream_status.restype = i
             L.fock_one_electron.argtypes = [ctypes.POINTER(fock_basis_desc), i, p, p, p, p, p, p]
@@ -293,6 +295,15 @@ def fock_work_stats(handle, D_host: np.ndarray, schwarz_thresh: float) -> dict:
     return {k: float(v) for k, v in zip(keys, out)}
 
 
+def fock_window_stats(handle, D_host: np.ndarray, schwarz_thresh: float) -> dict:
+    """Quartets and modelled operations by the arithmetic that evaluates them."""
+    D_host = np.ascontiguousarray(D_host, dtype=np.float64)
+    out = np.zeros(6)
+    _check(lib().fock_window_stats(handle, _np_ptr(D_host), float(schwarz_thresh), _np_ptr(out)), "fock_window_stats")
+    keys = ["quartets_fp64", "quartets_two_float", "quartets_fp32", "flops_fp64", "flops_two_float", "flops_fp32"]
+    return {k: float(v) for k, v in zip(keys, out)}
+
+
 def fock_stream_status(stream=None) -> int:
     return int(lib().fock_stream_status(_stream_handle(stream)))
 
@@ -482,6 +493,9 @@ class JKBuilder:
 
     def stats(self, D_host, tau=None) -> dict:
         return fock_work_stats(self.handle, D_host, self.tau if tau is None else tau)
+
+    def window_stats(self, D_host, tau=None) -> dict:
+        return fock_window_stats(self.handle, D_host, self.tau if tau is None else tau)
 
     def close(self):
         if getattr(self, "handle", None) is not None and self.handle.value:
