@@ -124,10 +124,8 @@ fock_status build_plan(const fock_shellpairs *const *bases, int nmol, BatchPlan 
     m.pf.insert(m.pf.end(), h.pf.begin(), h.pf.end());
     m.paf.insert(m.paf.end(), h.paf.begin(), h.paf.end());
     m.pal.insert(m.pal.end(), h.pal.begin(), h.pal.end());
-    m.U.insert(m.U.end(), h.U.begin(), h.U.end());
     m.Gp.insert(m.Gp.end(), h.Gp.begin(), h.Gp.end());
     m.Gpf.insert(m.Gpf.end(), h.Gpf.begin(), h.Gpf.end());
-    m.Uf.insert(m.Uf.end(), h.Uf.begin(), h.Uf.end());
     for (int o : h.eoff) m.eoff.push_back(o + (int)evals);
     m.E.insert(m.E.end(), h.E.begin(), h.E.end());
     m.Ef.insert(m.Ef.end(), h.Ef.begin(), h.Ef.end());

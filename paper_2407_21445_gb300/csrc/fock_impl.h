@@ -86,7 +86,6 @@ struct DevPairs {
   // primitive pairs
   const PZ *pz;        // (Px, Py, Pz, zeta)
   const float4 *pf;    // the same in FP32 (grid indices, seeds)
-  const double *U;     // U_P sqrt(zeta) (2/sqrt(pi))^(1/2), already folded into E (kept for reference)
   const int *eoff;     // offset of the primitive pair's E block
   const double *E;     // Hermite coefficients (Cartesian normalisation and U folded in)
   const double *Gp;    // primitive Schwarz factor G_[ab]; each pair's primitives sorted by it, descending
@@ -97,8 +96,7 @@ struct DevPairs {
   const float4 *paf;   // (P - A, zeta) with A the first shell of the canonical pair
   const float4 *pal;   // remainders of paf (two-float path): P - A and zeta less their FP32 values
   const float2 *E2;    // Hermite coefficients as two floats (null without the two-float path)
-  const float *Uf;     // U as above, FP32
-  const float *Ef;     // Hermite coefficients, FP32
+  const float *Ef;     // Hermite coefficients, FP32 (null without an FP32 path)
   const int *smol;     // shell -> molecule of a batch (null for one molecule)
   const int *satom;    // shell -> atom (shells on one atom share an index)
   const float *Gn;     // nshell^2: n_z G_xz for kept pairs (x, z), else 0 (GDG bound)
@@ -130,13 +128,12 @@ struct Staging {
   std::vector<int> cls;
   std::vector<PZ> pz;
   std::vector<float4> pf;
-  std::vector<double> U;
   std::vector<int> eoff;
   std::vector<double> E;
   std::vector<double> Gp;
   std::vector<float> Gpf;
   std::vector<float4> paf, pal;
-  std::vector<float> Uf, Ef, Gf, shl;
+  std::vector<float> Ef, Gf, shl;
   std::vector<int> smol;
   std::vector<int> satom;
   std::vector<float2> sRG;
