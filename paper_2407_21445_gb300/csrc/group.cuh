@@ -428,7 +428,7 @@ __device__ __forceinline__ void quartet_group(const KArgs &a, const Dims &d, con
   for (int i = gl; i < sl.y; i += G) scr[i] = 0.0f;  // zero ERIs
   const int2 pb = dp.prim[P], pk = dp.prim[Q];
   const int sip = bra_split(a.nsplit, pb.y), sjq = a.nsplit / sip;  // this group's share
-  const PrimScreen ps = prim_screen<true>(a, mv, sA, sB, sC, sD);
+  const PrimScreen ps = prim_screen(a, mv, sA, sB, sC, sD);
   const CentreDiff<PREC> ac = centre_diff<PREC>(dp, sA, sC);
   bool any = false;
   for (int ip = pb.x + (part & (sip - 1)); ip < pb.x + pb.y; ip += sip) {
@@ -655,7 +655,7 @@ __device__ __forceinline__ void run_group_list(const KArgs &a, int *counter, con
       if (i < end) {
         const MolView mv = mol_view(a, ab.x);
         const int2 cd = a.dp.ab[Q];
-        const float b = quartet_bound<true>(a, mv, ab.x, ab.y, cd.x, cd.y, P, Q);
+        const float b = quartet_bound(a, mv, ab.x, ab.y, cd.x, cd.y, P, Q);
         if (b >= 0.0f && share_used(a, P, Q, part)) {
           const QuartetWindows w = quartet_windows(a, mv, ab.x, ab.y, cd.x, cd.y, P, Q, b);
           in = PREC == kF64 ? w.f64 : (PREC == kFF ? w.ff : w.f32);

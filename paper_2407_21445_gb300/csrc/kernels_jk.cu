@@ -40,9 +40,6 @@ static float *s_boysf[64];
 static float2 *s_boysff[64];
 static ClassTables *s_tabs[64];
 
-
-
-
 // Shell-block maxima |D| (Sec. 3.2 density screening) and a finiteness check.
 __global__ void k_dprep(const double *__restrict__ D, int N, const int *__restrict__ sbf,
                         const int *__restrict__ sl, int ns, double *__restrict__ Dsh, float *__restrict__ Df,

@@ -33,8 +33,6 @@ void normalised_coefs(const fock_basis_desc *d, int s, double *out);
 
 namespace {
 
-constexpr int kMaxGroups = (LMAX + 1) * MAXPRIM;  // (angular momentum, contraction) kinds of shells
-
 // Workspace of the per-primitive values: a class that needs more is done in
 // pieces of whole shell pairs, a million threads each at least for s and p.
 constexpr long long kPieceDoubles = 64ll << 20;  // 512 MiB

@@ -79,40 +79,35 @@ __global__ void __launch_bounds__(128) k_schwarz_thread(SchwarzArgs a) {
 
 static_assert(sizeof(ClassTables) % 16 == 0, "the scratch behind the tables is aligned");
 
-__device__ __forceinline__ void group_sync(unsigned mask, int G) {
-  if (G > 1) __syncwarp(mask);
-}
-
-// R^{(0)}_{tuv}, t+u+v <= L, into the returned buffer (one of R0/R1).
+// R^{(0)}_{tuv}, t+u+v <= L, into the returned buffer (one of R0/R1), by one warp.
 // F must hold base values pref (-2alpha)^n F_n(T), n = 0..L; R0[0] = F[L].
 __constant__ double c_small[16] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15};
-template <int G, class Real>
-__device__ __forceinline__ Real *hermite_r(const ClassTables &ct, int L, Real X, Real Y, Real Z, const Real *F,
-                                           Real *R0, Real *R1, int gl, unsigned gmask) {
-  Real *cur = R0, *nxt = R1;
+__device__ __forceinline__ double *hermite_r_warp(const ClassTables &ct, int L, double X, double Y, double Z,
+                                                  const double *F, double *R0, double *R1, int lane) {
+  double *cur = R0, *nxt = R1;
   for (int n = L - 1; n >= 0; --n) {
-    int cnt = nherm(L - n);
-    for (int e = gl; e < cnt; e += G) {
-      Real v;
+    const int cnt = nherm(L - n);
+    for (int e = lane; e < cnt; e += 32) {
+      double v;
       if (e == 0) {
         v = F[n];
       } else {
-        int t = ct.hvec[e][0], u = ct.hvec[e][1], w = ct.hvec[e][2];
+        const int t = ct.hvec[e][0], u = ct.hvec[e][1], w = ct.hvec[e][2];
         if (t > 0) {
           v = X * cur[hidx(t - 1, u, w)];
-          if (t > 1) v = fma((Real)c_small[t - 1], cur[hidx(t - 2, u, w)], v);
+          if (t > 1) v = fma(c_small[t - 1], cur[hidx(t - 2, u, w)], v);
         } else if (u > 0) {
           v = Y * cur[hidx(t, u - 1, w)];
-          if (u > 1) v = fma((Real)c_small[u - 1], cur[hidx(t, u - 2, w)], v);
+          if (u > 1) v = fma(c_small[u - 1], cur[hidx(t, u - 2, w)], v);
         } else {
           v = Z * cur[hidx(t, u, w - 1)];
-          if (w > 1) v = fma((Real)c_small[w - 1], cur[hidx(t, u, w - 2)], v);
+          if (w > 1) v = fma(c_small[w - 1], cur[hidx(t, u, w - 2)], v);
         }
       }
       nxt[e] = v;
     }
-    group_sync(gmask, G);
-    Real *tmp = cur;
+    __syncwarp();
+    double *tmp = cur;
     cur = nxt;
     nxt = tmp;
   }
@@ -144,9 +139,9 @@ __global__ void __launch_bounds__(128) k_schwarz_warp(SchwarzArgs a, int la, int
   double acc[4] = {0.0, 0.0, 0.0, 0.0}, pm = 0.0;
   for (int j = i; j < pr.x + pr.y; ++j) {
     const PrimQuartet q = prim_quartet(P4, Pf, dp.pz[j], dp.pf[j]);
-    boys_seeds_rt<32>(a.boys, q, L, F, R0, lane);
+    boys_seeds_warp(a.boys, q, L, F, R0, lane);
     __syncwarp();
-    const double *R = hermite_r<32>(ct, L, q.X, q.Y, q.Z, F, R0, R1, lane, 0xffffffffu);
+    const double *R = hermite_r_warp(ct, L, q.X, q.Y, q.Z, F, R0, R1, lane);
     for (int k = 0; k < 4; ++k) {
       const int kc = lane + 32 * k;
       if (kc >= nab) break;
