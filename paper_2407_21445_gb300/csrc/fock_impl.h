@@ -256,12 +256,18 @@ struct ScratchLayout {
          total = 0;
 };
 ScratchLayout scratch_layout(const fock_shellpairs *sp);
+// FOCK_OK, or what a build answers to its arguments.  (api.cu)
+fock_status check_build_args(const fock_shellpairs *sp, const double *D, double schwarz_thresh, const double *J,
+                             const double *K);
+// The work of one build with its scratch in place, whatever it holds; ev (may be
+// null): tiers + 1 events, recorded around the tiers, which then run one after
+// the other.  Under a RelaxedCaptureMode.  (api.cu)
+fock_status enqueue_build(const fock_shellpairs *sp, const double *D, double schwarz_thresh, double *J, double *K,
+                          char *scratch, cudaStream_t stream, const cudaEvent_t *ev);
 
 // Status of a CUDA runtime result; a failure also sets the text returned by
 // fock_last_error ("where: error name (description)").  (api.cu)
 fock_status cuda_status(cudaError_t e, const char *where);
-// FOCK_SYNC_CHECK=1 in the environment: synchronise after every launch.
-bool sync_each_launch();
 
 // host helpers (host_pairs.cpp)
 const ClassTables &class_tables();

@@ -230,23 +230,14 @@ __device__ __forceinline__ ff boys_one_ff(const float2 *__restrict__ tab, ff T, 
     const int gi = __float2int_rn(T.h * BOYSFF_INVH);
     const float2 *row = tab + (size_t)gi * BOYSFF_NORD + m;
     const float2 g0 = __ldg(row), g1 = __ldg(row + 1), g2 = __ldg(row + 2);
-    const float g3 = __ldg(row + 3).x, g4 = __ldg(row + 4).x, g5 = __ldg(row + 5).x;
-    const ff x = ff_two(__fsub_rn((float)gi * (1.0f / BOYSFF_INVH), T.h), -T.l);
-    ff y2 = ff_sqr(x);
-    y2 = {0.5f * y2.h, 0.5f * y2.l};
-    const float y3 = x.h * y2.h * (1.0f / 3.0f), y4 = x.h * y3 * 0.25f, y5 = x.h * y4 * 0.2f;
-    const ff p1 = ff_mul(x, {g1.x, g1.y}), p2 = ff_mul(y2, {g2.x, g2.y});
-    const float t = fmaf(y5, g5, fmaf(y4, g4, y3 * g3));
-    const ff s1 = ff_fast2(g0.x, p1.h), s2 = ff_fast2(s1.h, p2.h);
-    const float lo = __fadd_rn(__fadd_rn(g0.y, __fadd_rn(p1.l, p2.l)), __fadd_rn(__fadd_rn(s1.l, s2.l), t));
-    return ff_fast2(s2.h, lo);
+    return boys_taylor_ff(boys_arg_ff(T, gi), {g0.x, g0.y}, {g1.x, g1.y}, {g2.x, g2.y}, __ldg(row + 3).x,
+                          __ldg(row + 4).x, __ldg(row + 5).x);
   }
   const ff rt = ff_norm(ff_rsqrt(T)), it = ff_norm(ff_sqr(rt));
-  ff f = ff_mul(ff{0.886226952f, -2.66231996e-8f}, rt);  // sqrt(pi)/2
-  for (int k = 1; k <= m; ++k) f = ff_norm(ff_mul(f, ff_mulf(it, k - 0.5f)));
+  ff f = boys_far0_ff(rt);
+  for (int k = 1; k <= m; ++k) f = boys_far_ff(f, it, k);
   return f;
 }
-
 
 // F_m(T) pref (-2 alpha)^m of one order, FP64 and FP32 (see boys_seeds,
 // boys_seeds_f32).
