@@ -602,7 +602,7 @@ __device__ __forceinline__ void quartet_group(const KArgs &a, const Dims &d, con
       v = f2d_any(f * (s0 + s1));
     } else {
       const ff s = ff_add(s0, s1);
-      v = f2d_any(f * s.h) + f2d_any(f * s.l);
+      v = f2d_any(f * s.h) + f2d_fin(f * s.l);  // l is finite where h is
     }
     atomicAdd((t.blk < 2 ? mv.J : mv.K) + place(t), v);
   }
