@@ -34,8 +34,9 @@ void normalised_coefs(const fock_basis_desc *d, int s, double *out);
 namespace {
 
 // Workspace of the per-primitive values: a class that needs more is done in
-// pieces of whole shell pairs, a million threads each at least for s and p.
-constexpr long long kPieceDoubles = 64ll << 20;  // 512 MiB
+// pieces of whole shell pairs, a million threads each at least for s and p;
+// where the device has not that much left, in smaller ones down to 64 KiB.
+constexpr long long kPieceDoubles = 64ll << 20, kMinPieceDoubles = 8ll << 10;  // 512 MiB
 
 // Shells of one kind, at perm[first ..].
 struct ShellGroup {
@@ -313,10 +314,10 @@ extern "C" fock_status fock_one_electron(const fock_basis_desc *desc, int32_t na
   };
   std::vector<GroupPair> gps;
   std::vector<ClassWork> work;
-  size_t buf_doubles = 0;
+  long long piece = kPieceDoubles;
   // primitive pairs of a class whose values the workspace holds at a time
-  auto piece_prims = [](const ClassWork &w) {
-    return std::max<long long>(MAXPRIM * MAXPRIM, kPieceDoubles / ((w.nsplit + 2) * ncart(w.la) * ncart(w.lb)));
+  auto piece_prims = [&piece](const ClassWork &w) {
+    return std::max<long long>(MAXPRIM * MAXPRIM, piece / ((w.nsplit + 2) * ncart(w.la) * ncart(w.lb)));
   };
   for (int la = 0; la <= LMAX; ++la)
     for (int lb = 0; lb <= la; ++lb) {
@@ -334,7 +335,6 @@ extern "C" fock_status fock_one_electron(const fock_basis_desc *desc, int32_t na
       if (w.npair == 0) continue;
       // few primitive pairs: share the nuclei, too, between up to 8 threads
       while (w.nsplit < 8 && 2 * w.nsplit <= natom && w.nprim * w.nsplit < kFillThreads) w.nsplit *= 2;
-      buf_doubles = std::max(buf_doubles, (size_t)((w.nsplit + 2) * ncart(la) * ncart(lb) * std::min(w.nprim, piece_prims(w))));
       work.push_back(w);
     }
   std::vector<double> ex(np_tot), cc(np_tot);
@@ -360,7 +360,15 @@ extern "C" fock_status fock_one_electron(const fock_basis_desc *desc, int32_t na
   const size_t o_z = add(Z, natom > 0 ? sizeof(double) * natom : 0);
   const size_t in_bytes = (host.size() + 255) & ~(size_t)255;
   char *d = nullptr;
-  e = cudaMallocAsync((void **)&d, in_bytes + buf_doubles * sizeof(double), stream);
+  for (;; piece /= 8) {
+    size_t buf_doubles = 0;
+    for (const ClassWork &w : work)
+      buf_doubles = std::max(buf_doubles, (size_t)((w.nsplit + 2) * ncart(w.la) * ncart(w.lb) *
+                                                   std::min(w.nprim, piece_prims(w))));
+    e = cudaMallocAsync((void **)&d, in_bytes + buf_doubles * sizeof(double), stream);
+    if (e != cudaErrorMemoryAllocation || piece <= kMinPieceDoubles) break;
+    cudaGetLastError();  // less may be left
+  }
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FOCK_ERR_OOM : FOCK_ERR_CUDA;
   e = cudaMemcpyAsync(d, host.data(), host.size(), cudaMemcpyHostToDevice, stream);
   OneArgs a{};

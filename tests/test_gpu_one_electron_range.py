@@ -40,3 +40,38 @@ def test_around_the_end_of_the_table(env):
     Z = np.arange(1.0, len(d) + 1)
     _, _, V = fk.fock_one_electron(bas, Z, xyz)
     assert np.abs(V.cpu().numpy() - oracle.nuclear(bas, Z, xyz)).max() < 1e-11
+
+
+def test_little_device_memory(env):
+    """A memory pool that ends at 32 MiB, set as the device's: the per-primitive
+    values of 200 contracted d shells (five times that) go in small pieces."""
+    import ctypes
+    torch, fk = env
+
+    class Props(ctypes.Structure):  # CUmemPoolProps
+        _fields_ = [("alloc_type", ctypes.c_int), ("handle_types", ctypes.c_int), ("loc_type", ctypes.c_int),
+                    ("loc_id", ctypes.c_int), ("security", ctypes.c_void_p), ("max_size", ctypes.c_size_t),
+                    ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
+
+    rng = np.random.Generator(np.random.PCG64(43))
+    bas = molgen.single_shell_basis([(2, rng.uniform(-6, 6, 3), rng.uniform(0.2, 4.0, 8), rng.uniform(0.2, 1.0, 8))
+                                     for _ in range(200)])
+    nuclei = rng.uniform(-6, 6, (2, 3))
+    ref = fk.fock_one_electron(bas, [1.0, 8.0], nuclei)
+    assert 20100 * 64 * 36 * 3 * 8 > 5 * (32 << 20)
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, old = ctypes.c_void_p(), ctypes.c_void_p()
+    dev = torch.cuda.current_device()
+    props = Props(alloc_type=1, loc_type=1, loc_id=dev, max_size=32 << 20)
+    torch.cuda.synchronize()
+    assert cu.cuDeviceGetMemPool(ctypes.byref(old), dev) == 0
+    assert cu.cuMemPoolCreate(ctypes.byref(pool), ctypes.byref(props)) == 0
+    assert cu.cuDeviceSetMemPool(dev, pool) == 0
+    try:
+        out = fk.fock_one_electron(bas, [1.0, 8.0], nuclei)
+        torch.cuda.synchronize()
+    finally:
+        assert cu.cuDeviceSetMemPool(dev, old) == 0
+        assert cu.cuMemPoolDestroy(pool) == 0
+    for a, b in zip(out, ref):
+        assert float(b.abs().max()) > 0 and float((a - b).abs().max()) <= 1e-13 * float(b.abs().max())
