@@ -207,10 +207,10 @@ inline void set_split(Tier &t) {
 // ends; but bodies that share an SM also evict one another's instructions, and in
 // a build large enough for the ends not to matter that costs more.  Measured, one
 // after the other against side by side, modelled operations of the build in
-// brackets: mixed C12H26 (0.3e11) 23.5 against 18.4 ms, C20H42 (1.2e11) 57.5
-// against 55.4, (H2O)20 (1.7e11) 69 against 75, (H2O)32 (7e11) 234 against 299,
-// (H2O)40 (13e11) 414 against 557; FP64 C20H42 104 against 100, C31H64 (3.1e11)
-// within 3 % either way, (H2O)32 446 against 491, (H2O)40 818 against 908.
+// brackets: mixed C12H26 (0.3e11) 22.5 against 17.9 ms, C20H42 (1.2e11) 55.4
+// against 54.3, (H2O)20 (1.7e11) 69 against 74, (H2O)32 (7e11) 222 against 284,
+// (H2O)40 (13e11) 403 against 549; FP64 C20H42 100 against 97, C31H64 (3.1e11)
+// 248 against 249, (H2O)32 416 against 462, (H2O)40 771 against 882.
 inline void set_queued(std::vector<Tier> &tiers, bool mixed) {
   double cost = 0.0;
   for (const Tier &t : tiers) cost += t.cost;

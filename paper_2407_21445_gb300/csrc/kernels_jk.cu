@@ -1,6 +1,6 @@
-// GB300 (sm_103a) kernels around the J/K quartet kernels: Schwarz factors,
-// density preparation and decay bound, symmetrisation, and the launches of a
-// class pair's quartet kernels (kernels_reg.cuh, kernels_group.cu).
+// GB300 (sm_103a) kernels around the J/K quartet kernels: density preparation and
+// decay bound, symmetrisation, and the launches of a class pair's quartet kernels
+// (kernels_reg.cuh, kernels_group.cu).
 //
 // Integral scheme: McMurchie-Davidson (arXiv:2407.21445 Sec. 4.1, Eqs. MD
 // def, EabP def1-3): a primitive quartet is

@@ -60,20 +60,16 @@ enum Epi {
 // (BF16 weights), on the tensor cores: a block of eight warps owns a 32 x 64 tile
 // of C (each warp 16 x 16), K in steps of 32, the operands of the next four
 // steps under way in registers while one is multiplied (K = 128: all of them from
-// the start; with four warps and one step ahead a training step at 4096 rows took
-// 211 us, so 196 us).  A is split
-// into a TF32 high part and a TF32 remainder whose products are both
-// accumulated in FP32, which keeps the product accurate to about FP32 rounding
-// (BF16 weights are exact in TF32).
+// the start).  A is split into a TF32 high part and a TF32 remainder whose
+// products are both accumulated in FP32, which keeps the product accurate to
+// about FP32 rounding (BF16 weights are exact in TF32).
 //
 // At the training sizes (4096 rows, 128 hidden units) the work is a few
 // microseconds of any unit's rate; what counts is blocks in flight, hidden load
-// latency and launches.  32-row tiles give 256 blocks where 64-row tiles gave
-// 128 for 152 SMs; loss and activation derivative ride along in the epilogues;
-// the three weight gradients with their bias sums are one launch (k_grads).
-// A training step at 4096 rows took 1.67 ms before (17 launches; 680 us of it
-// the bias sums, one thread per column, and 1.47 ms under the profiler the
-// weight gradients on 4 to 8 blocks); now 0.20 ms
+// latency and launches.  32-row tiles give 256 blocks for 152 SMs, 64-row tiles
+// 128; loss and activation derivative ride along in the epilogues; the three weight
+// gradients with their bias sums are one launch (k_grads).  A training step at
+// 4096 rows takes 0.20 ms, with four warps and one step ahead 15 us more.
 constexpr int BM = 32, BN = 64, GK = 32, GTHREADS = 256, GDEPTH = 4;
 struct GemmArgs {
   int M, N, K, lda, ldb, ldc;
@@ -204,10 +200,10 @@ __global__ void __launch_bounds__(GTHREADS) k_gemm(GemmArgs g) {
 // mma, 12 conversions, loads) bounds the kernel, so nothing else stands in the
 // chain and every scheduler has a warp of its own: the operands come from L2
 // straight into registers, GAHEAD steps ahead, without shared memory or barriers,
-// and the tile is the smallest that the instruction has.  A training step at 4096
-// rows and 128 hidden units: 243 us with 32 x 32 tiles behind a four-stage cp.async
-// pipeline, 211 us so (GAHEAD = 8: 223 us; all loads of eight steps in one go
-// and two buffers: 5 us more than one by one).
+// and the tile is the smallest that the instruction has.  Against it, in a training
+// step at 4096 rows and 128 hidden units: 32 x 32 tiles behind a four-stage cp.async
+// pipeline 32 us more, GAHEAD = 8 12 us more, all loads of eight steps in one go
+// into two buffers 5 us more than one by one.
 constexpr int GTM = 16, GTN = 32, GAHEAD = 16;
 struct GradLayer {
   const float *d, *x;  // [rows][M], [rows][N]

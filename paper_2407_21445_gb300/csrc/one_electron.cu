@@ -14,10 +14,10 @@
 // Cartesian pair; a second kernel adds up the primitive pairs of each element in
 // a fixed order and writes both triangles.  The nuclei are the inner loop and
 // carry nearly all the work, about 16 (ss) to 250 (dd) FP64 operations each, so
-// the kernel is bound by the FP64 pipe.  One thread per (ordered shell pair,
-// Cartesian pair), as before, repeated the Boys function and the recursion for
-// each of up to 36 (dd) Cartesian pairs and both orders in local memory: 165 ms
-// for (H2O)32 (608 functions, 96 nuclei); now 2.4 ms (call included).
+// the kernel is bound by the FP64 pipe: 2.4 ms for (H2O)32 (608 functions, 96
+// nuclei; call included), 1.2 ms of it the pipe's by the operation model.  A thread
+// per Cartesian pair and order instead repeats the Boys function and the
+// recursion up to 72 times (165 ms).
 #include <math.h>
 #include <string.h>
 

@@ -7,10 +7,10 @@
 // after it twice -- is one item of work: one thread with everything in
 // registers for the classes up to la + lb = 2, one warp with the Hermite
 // integrals in shared memory for the others.  The rows' sums are added up in
-// order by a last kernel.  The rows make the parallel work: with one warp per
-// pair walking all n^2 primitive quartets of a contracted pair (up to 4096), the
-// longest pairs' latency was the kernel's time: 3.1 ms for C12H26, 7 ms for a
-// triple-zeta ethane; now 0.65 ms for C12H26.
+// order by a last kernel.  The rows make the parallel work: 0.65 ms for C12H26.
+// One warp per pair that walks all n^2 primitive quartets of a contracted pair (up
+// to 4096) takes the longest pair's latency instead: 3.1 ms, 7 ms for a
+// triple-zeta ethane.
 #include <algorithm>
 
 #include "kernels_reg.cuh"

@@ -38,8 +38,9 @@ struct RelaxedCaptureMode {
 // A set for one build on `user`, or null when the build has to stay on that one
 // stream: it is being captured, or every set is still busy with builds of other
 // streams (sharing a set with another stream's unfinished build would order
-// two streams that the caller keeps independent).  Called under a
-// RelaxedCaptureMode.
+// two streams that the caller keeps independent).  On one stream the launches
+// follow one another: C20H42 83 against 72 ms (mixed 43 against 41), three waters
+// 4.7 against 1.2 ms.  Called under a RelaxedCaptureMode.
 StreamSet *lease_streams(cudaStream_t user);
 void return_streams(StreamSet *set);
 
