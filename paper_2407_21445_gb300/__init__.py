@@ -23,12 +23,12 @@ optionally atom, as produced by molgen.make_basis):
 The SCF driver (scf.RHF, scf.sad_guess) and the learned initial density
 (guess.LearnedGuess.load(".../guess_mlp.npz")) build on the same library.
 """
-from .fock import (FOCK_FP64, FOCK_MIXED, MLP, NCLASS, FockError, JKBuilder, fock_autotune, fock_boys_host,
+from .fock import (FOCK_FP64, FOCK_MIXED, FOCK_NO_TWO_FLOAT, MLP, NCLASS, FockError, JKBuilder, fock_autotune, fock_boys_host,
                    fock_boys_table_info, fock_build_jk, fock_build_jk_batched, fock_hermite_count, fock_hermite_e, fock_kernels_per_build, fock_nbasis, fock_one_electron,
                    fock_shellpairs_build, fock_shellpairs_free, fock_status_string, fock_stream_status,
                    fock_work_stats, lib, make_opts, schedule_of)
 
-__all__ = ["FOCK_FP64", "FOCK_MIXED", "MLP", "NCLASS", "FockError", "JKBuilder", "fock_autotune", "fock_boys_host", "fock_boys_table_info",
+__all__ = ["FOCK_FP64", "FOCK_MIXED", "FOCK_NO_TWO_FLOAT", "MLP", "NCLASS", "FockError", "JKBuilder", "fock_autotune", "fock_boys_host", "fock_boys_table_info",
            "fock_build_jk", "fock_build_jk_batched", "fock_hermite_count", "fock_hermite_e", "fock_kernels_per_build", "fock_nbasis", "fock_one_electron",
            "fock_shellpairs_build", "fock_shellpairs_free", "fock_status_string", "fock_stream_status",
            "fock_work_stats", "lib", "make_opts", "schedule_of"]

@@ -26,8 +26,6 @@ def workload_key(bases, schwarz_thresh: float, opts: fock.fock_opts | None, devi
     desc = {"gpu": device_name, "precision": int(o.precision), "fp32_cutoff": float(o.fp32_cutoff),
             "prune_eps": float(o.prune_eps), "warp_scratch": int(o.warp_scratch), "reg_max_L": int(o.reg_max_L),
             "tau": float(schwarz_thresh), "molecules": comp}
-    if o.two_float != 0:  # the default's keys stay what they were
-        desc["two_float"] = int(o.two_float)
     return hashlib.sha1(json.dumps(desc, sort_keys=True).encode()).hexdigest()
 
 

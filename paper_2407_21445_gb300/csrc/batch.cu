@@ -79,7 +79,6 @@ bool same_opts(const fock_shellpairs *a, const fock_shellpairs *b) {
          a->opts.fp32_cutoff == b->opts.fp32_cutoff && a->opts.prune_eps == b->opts.prune_eps &&
          a->opts.group_override == b->opts.group_override && a->opts.warp_scratch == b->opts.warp_scratch &&
          a->opts.reg_max_L == b->opts.reg_max_L && a->opts.tune_isolate == b->opts.tune_isolate &&
-         a->opts.two_float == b->opts.two_float &&
          memcmp(a->opts.schedule, b->opts.schedule, sizeof(a->opts.schedule)) == 0 && a->device == b->device;
 }
 
@@ -87,7 +86,7 @@ fock_status build_plan(const fock_shellpairs *const *bases, int nmol, BatchPlan 
   BatchPlan *bp = new BatchPlan();
   bp->nmol = nmol;
   bp->device = bases[0]->device;
-  bp->mixed = bases[0]->opts.precision == FOCK_MIXED && bases[0]->opts.fp32_cutoff > 0.0;
+  bp->mixed = mixed_opts(bases[0]->opts);
   bp->cutoff = bases[0]->opts.fp32_cutoff;
   bp->prim_eps = bases[0]->prune_eps;
   Staging m;

@@ -14,6 +14,11 @@
 
 namespace fk {
 
+// Whether a handle's quartets below the cutoff run in FP32.
+inline bool mixed_opts(const fock_opts &o) {
+  return (o.precision & ~FOCK_NO_TWO_FLOAT) == FOCK_MIXED && o.fp32_cutoff > 0.0;
+}
+
 constexpr int LMAX = 3;             // f functions
 constexpr int LTOT = 4 * LMAX;      // largest total angular momentum of a quartet
 constexpr int NCLASS = 10;          // pair classes (la >= lb)

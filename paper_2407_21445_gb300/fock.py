@@ -16,7 +16,7 @@ import numpy as np
 from . import _build
 
 FOCK_OK = 0
-FOCK_FP64, FOCK_MIXED = 0, 1
+FOCK_FP64, FOCK_MIXED, FOCK_NO_TWO_FLOAT = 0, 1, 0x100
 STATUS_NAMES = ["FOCK_OK", "FOCK_ERR_INVALID_ARG", "FOCK_ERR_UNSUPPORTED_L", "FOCK_ERR_NONFINITE",
                 "FOCK_ERR_OOM", "FOCK_ERR_CUDA", "FOCK_ERR_TIMEOUT", "FOCK_ERR_NOT_CONVERGED"]
 
@@ -41,7 +41,7 @@ class fock_opts(ctypes.Structure):
     _fields_ = [("precision", ctypes.c_int32), ("fp32_cutoff", ctypes.c_double), ("prune_eps", ctypes.c_double),
                 ("group_override", ctypes.c_int32), ("warp_scratch", ctypes.c_int32), ("reg_max_L", ctypes.c_int32),
                 ("tune_isolate", ctypes.c_int32), ("schedule", ctypes.c_int8 * (NCLASS * NCLASS)),
-                ("k_mode", ctypes.c_int32), ("k_thresh", ctypes.c_double), ("two_float", ctypes.c_int32)]
+                ("k_mode", ctypes.c_int32), ("k_thresh", ctypes.c_double)]
 
 
 _lock = threading.Lock()
@@ -183,12 +183,11 @@ class _BasisArrays:
 def make_opts(precision=FOCK_FP64, fp32_cutoff=1e-5, prune_eps=1e-3, group_override=0, warp_scratch=0,
               reg_max_L=0, schedule=None, k_mode=0, k_thresh=5e-6, two_float=True) -> fock_opts:
     o = fock_opts()
-    o.two_float = 0 if two_float else -1
     o.k_mode = k_mode
     o.k_thresh = k_thresh
     o.reg_max_L = reg_max_L
     o.warp_scratch = warp_scratch
-    o.precision = precision
+    o.precision = precision if two_float else precision | FOCK_NO_TWO_FLOAT
     o.fp32_cutoff = fp32_cutoff
     o.prune_eps = prune_eps
     o.group_override = group_override

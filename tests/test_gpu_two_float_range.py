@@ -157,7 +157,7 @@ def test_large_density_element_far_away(env):
 
 
 def test_window_turned_off(env):
-    """two_float = -1: no launch of its own for two floats, and the same J and K."""
+    """FOCK_NO_TWO_FLOAT: no launch of its own for two floats, and the same J and K."""
     torch, fk = env
     p = molgen.problem(0)
     b = [fk.JKBuilder(p.basis, p.tau, fk.make_opts(two_float=t)) for t in (True, False)]
@@ -167,11 +167,9 @@ def test_window_turned_off(env):
     assert float((J0 - J1).abs().max()) <= 1e-10 and float((K0 - K1).abs().max()) <= 1e-10
     with pytest.raises(fk.FockError):  # one choice per batch
         fk.fock_build_jk_batched([x.handle for x in b], [D, D], p.tau, [J0, J1], [K0, K1])
-    for v in (1, -2):
-        o = fk.make_opts()
-        o.two_float = v
+    for v in (2, 0x102, 0x200, -1):
         with pytest.raises(fk.FockError):
-            fk.JKBuilder(p.basis, p.tau, o)
+            fk.JKBuilder(p.basis, p.tau, fk.make_opts(precision=v))
     for x in b:
         x.close()
 
